@@ -45,98 +45,6 @@
 namespace tsvd {
 namespace {
 
-constexpr int TM = 64, TN = 64, TK = 16;
-
-__device__ __forceinline__ float2 cload(const float2* p, int64_t o, int conj) {
-  float2 v = p[o];
-  if (conj) v.y = -v.y;
-  return v;
-}
-
-// C = op(A) op(B), batched, generic strides (see CGemm in tsvd_internal.h).  64 x 64 tile per
-// CTA, 4 x 4 complex outputs per thread; operand tiles staged through shared memory with
-// threads running along whichever index is contiguous in global memory.
-__global__ void __launch_bounds__(256) cgemm_fp32_kernel(CGemm g) {
-  __shared__ float2 As[TK][TM + 1];
-  __shared__ float2 Bs[TK][TN + 1];
-  if (g.kdev) {
-    const int kk = *g.kdev;
-    if (g.dynM) g.M = kk;
-    if (g.dynN) g.N = kk;
-    if (g.dynK) g.K = kk;
-  }
-  if ((int)blockIdx.x * TM >= g.M || (int)blockIdx.y * TN >= g.N) return;
-  const int bz = blockIdx.z;
-  const float2* A = g.a.p + (int64_t)(g.a.idx ? g.a.idx[bz] : bz) * g.a.bs;
-  const float2* B = g.b.p + (int64_t)(g.b.idx ? g.b.idx[bz] : bz) * g.b.bs;
-  float2* C = const_cast<float2*>(g.c.p) + (int64_t)(g.c.idx ? g.c.idx[bz] : bz) * g.c.bs;
-  const int i0 = blockIdx.x * TM, j0 = blockIdx.y * TN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const bool a_rows = g.a.s0 == 1;
-  const bool b_ctr = g.b.s0 == 1;
-  float accr[4][4], acci[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) accr[r][c] = acci[r][c] = 0.f;
-  for (int l0 = 0; l0 < g.K; l0 += TK) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = tid + 256 * u;
-      int ii, ll;
-      if (a_rows) {
-        ii = e % TM;
-        ll = e / TM;
-      } else {
-        ll = e % TK;
-        ii = e / TK;
-      }
-      int i = i0 + ii, l = l0 + ll;
-      As[ll][ii] = (i < g.M && l < g.K) ? cload(A, i * g.a.s0 + l * g.a.s1, g.a.conj)
-                                         : make_float2(0.f, 0.f);
-      int jj;
-      if (b_ctr) {
-        ll = e % TK;
-        jj = e / TK;
-      } else {
-        jj = e % TN;
-        ll = e / TN;
-      }
-      const int j = j0 + jj;
-      l = l0 + ll;
-      Bs[ll][jj] = (j < g.N && l < g.K) ? cload(B, l * g.b.s0 + j * g.b.s1, g.b.conj)
-                                         : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int l = 0; l < TK; ++l) {
-      float2 a[4], b[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[l][ty + 16 * r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[l][tx + 16 * c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          accr[r][c] = fmaf(a[r].x, b[c].x, fmaf(-a[r].y, b[c].y, accr[r][c]));
-          acci[r][c] = fmaf(a[r].x, b[c].y, fmaf(a[r].y, b[c].x, acci[r][c]));
-        }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = i0 + ty + 16 * r;
-    if (i >= g.M) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int j = j0 + tx + 16 * c;
-      if (j < g.N) C[i * g.c.s0 + j * g.c.s1] = make_float2(accr[r][c], acci[r][c]);
-    }
-  }
-}
-
 // (hi, lo) -= ax^2 + ay^2 in double-single arithmetic: the squares are split exactly with
 // FMA, the sums are two-sums (the _rn intrinsics keep the compiler from contracting them).
 __device__ __forceinline__ void ds_sub_norm2(float& hi, float& lo, float ax, float ay) {
@@ -922,13 +830,6 @@ size_t cholqr_smem(int k) {
          (size_t)k * sizeof(float2) + (size_t)k * sizeof(float) + (size_t)k * sizeof(int);
 }
 
-cudaError_t gemm_fp32(const CGemm& g, cudaStream_t st) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
-  dim3 grid((g.M + TM - 1) / TM, (g.N + TN - 1) / TN, g.batch);
-  cgemm_fp32_kernel<<<grid, 256, 0, st>>>(g);
-  return cudaGetLastError();
-}
-
 CMat mat(const float2* p, const int* idx, int64_t bs, int64_t s0, int64_t s1, int conj = 0) {
   CMat m;
   m.p = p;
@@ -955,7 +856,7 @@ CGemm gemm(int M, int N, int K, int batch, const CMat& a, const CMat& b, const C
 }  // namespace
 
 cudaError_t launch_cgemm(const CGemm& g, int engine, cudaStream_t st) {
-  if (engine == RSVT_GEMM_FP32) return gemm_fp32(g, st);
+  if (engine == RSVT_GEMM_FP32) return launch_cgemm_fp32(g, st);
   return launch_cgemm_tc(g, engine, st);
 }
 

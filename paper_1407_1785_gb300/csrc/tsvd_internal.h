@@ -326,6 +326,7 @@ struct CGemm {
 enum RsvtEngine : int { RSVT_GEMM_FP32 = 0, RSVT_GEMM_TF32 = 1, RSVT_GEMM_BF16 = 2,
                         RSVT_GEMM_3XTF32 = 3 };
 cudaError_t launch_cgemm(const CGemm& g, int engine, cudaStream_t st);
+cudaError_t launch_cgemm_fp32(const CGemm& g, cudaStream_t st);
 cudaError_t launch_cgemm_tc(const CGemm& g, int engine, cudaStream_t st);
 // Number of tensor-core product launches whose bounded waits expired since the last call
 // (reset to 0); waits for `st`.
