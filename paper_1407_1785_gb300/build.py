@@ -19,9 +19,10 @@ BUILD_DIR = os.path.join(PKG, "_build")
 LIB_DIR = os.path.join(PKG, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libtsvd.so")
 
-SOURCES = ["tsvd_api.cu", "tube_pass.cu", "slice_svt.cu", "tsvd_noalloc.cu", "rsvt.cu",
+SOURCES = ["tsvd_api.cu", "tube_pass.cu", "slice_svt.cu", "slice_g8.cu", "slice_g16.cu",
+           "slice_g32.cu", "slice_batch.cu", "tsvd_noalloc.cu", "rsvt.cu",
            "tc_gemm.cu", "fp32_gemm.cu", "factor.cu", "peak_probe.cu"]
-HEADERS = ["tsvd_internal.h", "tube_tile.cuh"]
+HEADERS = ["tsvd_internal.h", "slice_svt.cuh", "slice_kernel.cuh", "tube_tile.cuh"]
 
 ARCH_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
