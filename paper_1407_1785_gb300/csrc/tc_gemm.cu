@@ -10,19 +10,26 @@
 //           hi*hi + hi*lo + lo*hi (the lo*lo term is below FP32 rounding), kind::tf32;
 //   BF16    operands rounded to BF16, kind::f16 with BF16 inputs, K = 16 per instruction.
 //
-// Work split.  One CTA (256 threads) per 128 x 64 tile of C and per batch entry.  The K
-// range is walked in chunks; for each chunk all threads load the complex operand tiles from
-// global memory (any strides, optional conjugation), form the real planes (re, im, re+im; hi
-// and lo for 3XTF32) and store them in the canonical no-swizzle K-major layout: 8-row x
-// 16-byte core matrices, consecutive 8-row groups 128 bytes apart (stride-dimension offset),
-// consecutive K core matrices one plane height apart (leading-dimension offset).  One
-// thread then issues the chunk's MMAs and commits them to the chunk buffer's mbarrier; two
-// chunk buffers alternate so loading chunk c+1 overlaps the MMAs of chunk c.  With 3XTF32
+// Work split.  One CTA per 128 x 64 tile of C and per batch entry: 384 threads that stage the
+// operands and one warp that issues the MMAs.  The K range is walked in chunks; for each chunk
+// the staging threads load the rows the operands have (any strides, optional conjugation),
+// form the real planes (re, im, re+im; hi and lo for 3XTF32) and store them in the canonical
+// no-swizzle K-major layout: 8-row x 16-byte core matrices, consecutive 8-row groups 128 bytes
+// apart (stride-dimension offset), consecutive K core matrices one plane height apart
+// (leading-dimension offset).  The last warp then issues the chunk's MMAs, on as many columns
+// as the tile has in steps of 16, and commits them to the chunk buffer's mbarrier; two chunk
+// buffers alternate so loading chunk c+1 overlaps the MMAs of chunk c.  With 3XTF32
 // each thread copies its share of the raw complex entries with cp.async into three private
 // slots, two chunks ahead, and converts chunk c from its slot: the global latency overlaps
 // two chunks of conversion and MMA issue instead of sitting in front of each chunk.  The epilogue
-// reads T1..T3 with tcgen05.ld (warp w reads TMEM lanes 32 (w mod 4) .. +31, i.e. its rows of
+// reads T1..T3 with tcgen05.ld (warp w < 8 reads TMEM lanes 32 (w mod 4) .. +31, i.e. its rows of
 // the tile, and half of the columns) and writes C.
+//
+// Bound by shared memory: a 3XTF32 chunk of 16 reads about 108 KB of planes for its 18 MMAs and
+// moves 120 KB through staging, ~1800 cycles at 128 B a cycle, of which a chunk now takes 2400.
+// With 256 threads that also issued the MMAs (18 x 64 cycles in front of one warp's conversion)
+// and staged whole tiles a chunk took 3100 (us, M x N x K, batch): 40 x 40 x 320, 31: 41 -> 27;
+// 320 x 40 x 240, 31: 31 -> 27; 352 x 80 x 288, 91: 146 -> 121; TF32 156 -> 96, BF16 128 -> 72.
 //
 // Every mbarrier wait is bounded; on expiry the kernel counts a timeout (read by the host
 // through tc_gemm_take_timeouts), waits again (bounded) for its own MMAs, frees its tensor
@@ -37,7 +44,8 @@ __device__ int g_tc_timeouts = 0;
 
 namespace {
 
-constexpr int BM = 128, BN = 64, NTHR = 256;
+constexpr int BM = 128, BN = 64;
+constexpr int NCONV = 384, NTHR = NCONV + 32;   // converting threads; with the warp that issues MMAs
 constexpr int TMEM_COLS = 256;     // >= 3 * BN fp32 accumulator columns, power of two
 constexpr long long kWaitIters = 1ll << 24;
 constexpr uint64_t kWaitNs = 2000000000ull;   // 2 s
@@ -120,9 +128,9 @@ __device__ __forceinline__ uint64_t now_ns() {
 }
 
 // Waits for the phase of parity `parity` of the mbarrier; false after kWaitNs or
-// kWaitIters polls, whichever comes first.
+// kWaitIters polls, whichever comes first (the clock is read from the 256th poll on).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const uint64_t t0 = now_ns();
+  uint64_t t0 = 0;
   for (long long it = 0; it < kWaitIters; ++it) {
     uint32_t done;
     asm volatile(
@@ -132,15 +140,25 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((it & 255) == 255 && now_ns() - t0 > kWaitNs) return false;
+    if ((it & 255) == 255) {
+      const uint64_t t = now_ns();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > kWaitNs) return false;
+    }
   }
   return false;
 }
 
-// 8-byte asynchronous global -> shared copy; with pred false it writes zeros and reads nothing.
-__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool pred) {
+// Asynchronous global -> shared copies of 8 and 16 bytes, of which `bytes` are read and the rest
+// written as zeros.
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(pred ? 8 : 0)
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(bytes)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
@@ -199,105 +217,132 @@ __device__ __forceinline__ void make_planes(const float2 (&x)[Cfg<ENG>::EPC], Ro
   }
 }
 
-// Loads and stores the planes of one operand tile (R rows x BK complex entries of chunk l0).
-// Row r of the tile is operand row row0 + r; entry (row, l) sits at base[row * sr + l * sl].
-template <int ENG, int R>
-__device__ __forceinline__ void stage_operand(unsigned char* planes, int plane_bytes,
-                                              const float2* base, int64_t sr, int64_t sl,
-                                              int conj, int row0, int nrows, int l0, int K) {
+// A converting thread's share of the two operand tiles (BM + BN rows x BK complex entries a chunk):
+// up to PER core-matrix rows, EPC consecutive entries along K of one tile row each; those of A
+// first.  Only rows the operands have are staged, spread over all threads: a row past them
+// feeds only outputs that are not stored, and a sketch or its Gram fills a fraction of a tile.
+// The addresses are worked out once and advance by a chunk per issue.
+template <int ENG>
+struct Share {
   using C = Cfg<ENG>;
-  constexpr int KG = Layout<ENG>::KG;
-  constexpr int ITEMS = R * KG;
-  constexpr int PER = ITEMS / NTHR;
-  static_assert(ITEMS % NTHR == 0, "tile items must divide the thread count");
-  float2 x[PER][C::EPC];
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int item = threadIdx.x + NTHR * u;
-    const int r = item % R, kg = item / R;
-    const int row = row0 + r;
-#pragma unroll
-    for (int q = 0; q < C::EPC; ++q) {
-      const int l = l0 + kg * C::EPC + q;
-      float2 v = make_float2(0.f, 0.f);
-      if (row < nrows && l < K) {
-        v = base[(int64_t)row * sr + (int64_t)l * sl];
-        if (conj) v.y = -v.y;
-      }
-      x[u][q] = v;
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int item = threadIdx.x + NTHR * u;
-    const int r = item % R, kg = item / R;
-    Row<ENG> row;
-    make_planes<ENG>(x[u], row);
-    const int off = (kg * (R / 8) + r / 8) * 128 + (r % 8) * 16;
-#pragma unroll
-    for (int pl = 0; pl < 3 * C::NSPLIT; ++pl) {
-      uint4 val;
-      val.x = row.w[pl][0];
-      val.y = row.w[pl][1];
-      val.z = row.w[pl][2];
-      val.w = row.w[pl][3];
-      *reinterpret_cast<uint4*>(planes + (size_t)pl * plane_bytes + off) = val;
-    }
-  }
-}
+  using L = Layout<ENG>;
+  static constexpr int PER = (BM + BN) * L::KG / NCONV;
+  static_assert((BM + BN) * L::KG % NCONV == 0, "tile items must divide the thread count");
+  const float2* src[PER];   // entry 0 of the item in the next chunk to issue
+  int64_t sl[PER];          // its stride along K
+  int off[PER];             // its place in a chunk buffer (plane 0), -1: no item
+  int pstep[PER];           // bytes from plane to plane
+  int k0[PER];              // its first entry within a chunk
+  bool conj[PER];
+  bool vec[PER];            // neighbours along K are 16-byte aligned pairs
 
-// Asynchronous copy of a thread's share of one operand tile (chunk l0) into its raw slots
-// raw[(u EPC + q) NTHR + tid]: the thread that converts an entry is the one that copied it,
-// so the copies need no barrier, only the thread's own cp.async.wait_group.
-template <int ENG, int R>
-__device__ __forceinline__ void issue_operand(float2* raw, const float2* base, int64_t sr,
-                                              int64_t sl, int row0, int nrows, int l0, int K) {
-  using C = Cfg<ENG>;
-  constexpr int PER = R * Layout<ENG>::KG / NTHR;
+  __device__ __forceinline__ void init(const CGemm& g, const float2* A, const float2* B, int i0,
+                                       int j0) {
+    const int ra = min(BM, g.M - i0), rb = min(BN, g.N - j0);
 #pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int item = threadIdx.x + NTHR * u;
-    const int r = item % R, kg = item / R;
-    const int row = row0 + r;
-#pragma unroll
-    for (int q = 0; q < C::EPC; ++q) {
-      const int l = l0 + kg * C::EPC + q;
-      const bool ok = row < nrows && l < K;
-      const float2* src = ok ? base + (int64_t)row * sr + (int64_t)l * sl : base;
-      cp_async8(raw + (size_t)(u * C::EPC + q) * NTHR + threadIdx.x, src, ok);
+    for (int u = 0; u < PER; ++u) {
+      int item = threadIdx.x + NCONV * u;
+      const bool is_a = item < ra * L::KG;
+      if (!is_a) item -= ra * L::KG;
+      const int rows = is_a ? ra : rb, kg = item / rows, r = item - kg * rows;
+      k0[u] = kg * C::EPC;
+      sl[u] = is_a ? g.a.s1 : g.b.s0;
+      conj[u] = (is_a ? g.a.conj : g.b.conj) != 0;
+      pstep[u] = is_a ? L::PLANE_A : L::PLANE_B;
+      const int place = (kg * ((is_a ? BM : BN) / 8) + r / 8) * 128 + (r % 8) * 16;
+      off[u] = kg >= L::KG ? -1 : is_a ? place : L::NPLANE * L::PLANE_A + place;
+      src[u] = (is_a ? A + (int64_t)(i0 + r) * g.a.s0 : B + (int64_t)(j0 + r) * g.b.s1) +
+               (int64_t)k0[u] * sl[u];
+      vec[u] = sl[u] == 1 && (reinterpret_cast<uintptr_t>(src[u]) & 15) == 0;
     }
   }
-}
 
-// Converts a thread's raw share into the planes (conjugating on the way).
-template <int ENG, int R>
-__device__ __forceinline__ void convert_operand(const float2* raw, int conj, unsigned char* planes,
-                                                int plane_bytes) {
-  using C = Cfg<ENG>;
-  constexpr int PER = R * Layout<ENG>::KG / NTHR;
+  __device__ __forceinline__ void advance() {
 #pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int item = threadIdx.x + NTHR * u;
-    const int r = item % R, kg = item / R;
-    float2 x[C::EPC];
+    for (int u = 0; u < PER; ++u) src[u] += C::BK * sl[u];
+  }
+
+  // The planes of item u from its complex entries.
+  __device__ __forceinline__ void store(int u, float2 (&x)[C::EPC], unsigned char* stage) const {
+    if (conj[u]) {
 #pragma unroll
-    for (int q = 0; q < C::EPC; ++q) {
-      x[q] = raw[(size_t)(u * C::EPC + q) * NTHR + threadIdx.x];
-      if (conj) x[q].y = -x[q].y;
+      for (int q = 0; q < C::EPC; ++q) x[q].y = -x[q].y;
     }
     Row<ENG> row;
     make_planes<ENG>(x, row);
-    const int off = (kg * (R / 8) + r / 8) * 128 + (r % 8) * 16;
 #pragma unroll
-    for (int pl = 0; pl < 3 * C::NSPLIT; ++pl) {
-      uint4 val;
-      val.x = row.w[pl][0];
-      val.y = row.w[pl][1];
-      val.z = row.w[pl][2];
-      val.w = row.w[pl][3];
-      *reinterpret_cast<uint4*>(planes + (size_t)pl * plane_bytes + off) = val;
+    for (int pl = 0; pl < L::NPLANE; ++pl)
+      *reinterpret_cast<uint4*>(stage + off[u] + pl * pstep[u]) =
+          make_uint4(row.w[pl][0], row.w[pl][1], row.w[pl][2], row.w[pl][3]);
+  }
+
+  // Chunk at l0 through registers.
+  __device__ __forceinline__ void load_store(int l0, int K, unsigned char* stage) {
+    float2 x[PER][C::EPC];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int left = off[u] < 0 ? 0 : K - l0 - k0[u];
+#pragma unroll
+      for (int q = 0; q < C::EPC; ++q)
+        x[u][q] = q < left ? src[u][q * sl[u]] : make_float2(0.f, 0.f);
+    }
+    advance();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      if (off[u] >= 0) store(u, x[u], stage);
+  }
+
+  // Asynchronous copy of the chunk at l0 into the thread's raw slots, pairs of entries at
+  // raw[(u EPC / 2 + q / 2) NCONV + tid]: the thread that converts an entry is the one that
+  // copied it, so the copies need no barrier, only the thread's own cp.async.wait_group.
+  // `any`: an address that can be read (entries past K copy nothing from it).
+  __device__ __forceinline__ void issue(float4* raw, int l0, int K, const float2* any) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      if (off[u] < 0) continue;
+      const int left = K - l0 - k0[u];
+#pragma unroll
+      for (int q = 0; q < C::EPC; q += 2) {
+        float4* dst = raw + (size_t)(u * C::EPC + q) / 2 * NCONV + threadIdx.x;
+        if (vec[u]) {
+          cp_async16(dst, q < left ? src[u] + q : any, max(0, min(2, left - q)) * 8);
+        } else {
+          float2* d2 = reinterpret_cast<float2*>(dst);
+          cp_async8(d2, q < left ? src[u] + q * sl[u] : any, q < left ? 8 : 0);
+          cp_async8(d2 + 1, q + 1 < left ? src[u] + (q + 1) * sl[u] : any, q + 1 < left ? 8 : 0);
+        }
+      }
+    }
+    advance();
+  }
+
+  // Converts the raw share into the planes.
+  __device__ __forceinline__ void convert(const float4* raw, unsigned char* stage) const {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      if (off[u] < 0) continue;
+      float2 x[C::EPC];
+#pragma unroll
+      for (int q = 0; q < C::EPC; q += 2) {
+        const float4 v = raw[(size_t)(u * C::EPC + q) / 2 * NCONV + threadIdx.x];
+        x[q] = make_float2(v.x, v.y);
+        x[q + 1] = make_float2(v.z, v.w);
+      }
+      store(u, x, stage);
     }
   }
+};
+
+// True in every converting thread when `bad` holds in one (named barrier 1).
+__device__ __forceinline__ bool conv_any(bool bad) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\n"
+      "barrier.cta.red.or.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)bad), "n"(NCONV)
+      : "memory");
+  return r != 0;
 }
 
 template <int ENG>
@@ -321,9 +366,8 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   const int i0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * L::STAGE + L::RAW);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 2 * L::STAGE + L::RAW + 32);
-  float2* raw = reinterpret_cast<float2*>(smem + 2 * L::STAGE);   // RAW_STAGES x (A, B)
-  auto raw_a = [&](int c) { return raw + (size_t)(c % 3) * ((L::RAW_A + L::RAW_B) / 8); };
-  auto raw_b = [&](int c) { return raw_a(c) + L::RAW_A / 8; };
+  float4* raw = reinterpret_cast<float4*>(smem + 2 * L::STAGE);   // RAW_STAGES x (A, B)
+  auto raw_of = [&](int c) { return raw + (size_t)(c % 3) * ((L::RAW_A + L::RAW_B) / 16); };
   const uint32_t bar0 = smem_u32(&bars[0]), bar1 = smem_u32(&bars[1]);
 
   if (warp == 0) {
@@ -342,58 +386,57 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)C::FMT << 7) | ((uint32_t)C::FMT << 10) |
-                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+  // columns of the instruction: those the tile has, in steps of 16
+  const int ncol = min(BN, (g.N - j0 + 15) / 16 * 16);
+  const uint32_t idesc = (1u << 4) | ((uint32_t)C::FMT << 7) | ((uint32_t)C::FMT << 10) |
+                         ((uint32_t)(ncol >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
   constexpr uint32_t LBO_A = (BM / 8) * 128, LBO_B = (BN / 8) * 128, SBO = 128;
   constexpr int KSTEPS = C::BK / C::KMMA;
   const int nk = (g.K + C::BK - 1) / C::BK;
   bool timed_out = false;
-  if constexpr (L::RAW_STAGES > 0) {
-    // chunks 0 and 1 in flight before the loop; one commit group per chunk (empty past nk)
+  const bool conv = tid < NCONV;   // the last warp issues the MMAs
+  Share<ENG> sh;
+  if (conv) {
+    sh.init(g, A, B, i0, j0);
+    if constexpr (L::RAW_STAGES > 0) {
+      // chunks 0 and 1 in flight before the loop; one commit group per chunk (empty past nk)
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      if (c < nk) {
-        issue_operand<ENG, BM>(raw_a(c), A, g.a.s0, g.a.s1, i0, g.M, c * C::BK, g.K);
-        issue_operand<ENG, BN>(raw_b(c), B, g.b.s1, g.b.s0, j0, g.N, c * C::BK, g.K);
+      for (int c = 0; c < 2; ++c) {
+        if (c < nk) sh.issue(raw_of(c), c * C::BK, g.K, A);
+        cp_async_commit();
       }
-      cp_async_commit();
     }
   }
   int kc = 0;
   for (; kc < nk; ++kc) {
     const int buf = kc & 1;
-    if constexpr (L::RAW_STAGES > 0) {
-      // chunk kc + 2 into the slot chunk kc - 1 used (converted by this thread last time)
-      if (kc + 2 < nk) {
-        issue_operand<ENG, BM>(raw_a(kc + 2), A, g.a.s0, g.a.s1, i0, g.M, (kc + 2) * C::BK, g.K);
-        issue_operand<ENG, BN>(raw_b(kc + 2), B, g.b.s1, g.b.s0, j0, g.N, (kc + 2) * C::BK, g.K);
-      }
-      cp_async_commit();
-    }
-    if (kc >= 2) {
-      const bool ok = mbar_wait(buf ? bar1 : bar0, (uint32_t)(((kc >> 1) - 1) & 1));
-      if (__syncthreads_or(!ok)) {
-        timed_out = true;
-        break;
-      }
-    }
     unsigned char* st = smem + (size_t)buf * L::STAGE;
-    unsigned char* pa = st;
-    unsigned char* pb = st + L::NPLANE * L::PLANE_A;
-    if constexpr (L::RAW_STAGES > 0) {
-      cp_async_wait<2>();   // this thread's copies of chunk kc have landed
-      convert_operand<ENG, BM>(raw_a(kc), g.a.conj, pa, L::PLANE_A);
-      convert_operand<ENG, BN>(raw_b(kc), g.b.conj, pb, L::PLANE_B);
-    } else {
-      const int l0 = kc * C::BK;
-      stage_operand<ENG, BM>(pa, L::PLANE_A, A, g.a.s0, g.a.s1, g.a.conj, i0, g.M, l0, g.K);
-      stage_operand<ENG, BN>(pb, L::PLANE_B, B, g.b.s1, g.b.s0, g.b.conj, j0, g.N, l0, g.K);
+    bool bad = false;
+    if (conv) {
+      if constexpr (L::RAW_STAGES > 0) {
+        // chunk kc + 2 into the slot chunk kc - 1 used (converted by this thread last time)
+        if (kc + 2 < nk) sh.issue(raw_of(kc + 2), (kc + 2) * C::BK, g.K, A);
+        cp_async_commit();
+      }
+      // the MMAs of chunk kc - 2 have read this buffer
+      bad = kc >= 2 && conv_any(!mbar_wait(buf ? bar1 : bar0, (uint32_t)(((kc >> 1) - 1) & 1)));
+      if (!bad) {
+        if constexpr (L::RAW_STAGES > 0) {
+          cp_async_wait<2>();   // this thread's copies of chunk kc have landed
+          sh.convert(raw_of(kc), st);
+        } else {
+          sh.load_store(kc * C::BK, g.K, st);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
+    if (__syncthreads_or(bad)) {
+      timed_out = true;
+      break;
+    }
+    if (tid == NCONV) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_base = smem_u32(pa), b_base = smem_u32(pb);
+      const uint32_t a_base = smem_u32(st), b_base = a_base + L::NPLANE * L::PLANE_A;
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
         const uint32_t d = tmem + (uint32_t)(p * BN);
@@ -429,7 +472,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   }
   const bool good = !timed_out && !__syncthreads_or(!ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (good && nk > 0) {
+  if (good && nk > 0 && warp < 8) {   // 4 row groups x 2 halves of the columns
     const int q = warp & 3, half = warp >> 2;
     const int i = i0 + 32 * q + lane;
 #pragma unroll
