@@ -44,6 +44,38 @@ bool pick_group(int ld, int prefer, int& G, int& cpl) {
 
 }  // namespace
 
+// The block schedule: which circle slot each CTA takes in each block round.  Every next pair
+// joins two CTAs that hold one of its blocks each, and every CTA holds two blocks, so the next
+// pairs are the edges of cycles over the CTAs; giving each CTA the edge it leaves a cycle by
+// lets every CTA keep one block and trade the other.  The rotations and their order are those
+// of the circle method, whichever CTA does them.
+static void fill_schedule(int C, unsigned char (*slot_of)[kMaxCtasPerSlice]) {
+  const int nb = 2 * C;
+  int at[2 * kMaxCtasPerSlice];   // CTA that holds a block
+  for (int r = 0; r < nb - 1; ++r) {
+    int bx[kMaxCtasPerSlice], by[kMaxCtasPerSlice], cta_of[kMaxCtasPerSlice];
+    for (int s = 0; s < C; ++s) {
+      round_robin_pair(r, s, nb, bx[s], by[s]);
+      cta_of[s] = r == 0 ? s : -1;
+    }
+    for (int c = 0; r > 0 && c < C; ++c) {
+      bool has = false;
+      for (int s = 0; s < C; ++s) has |= cta_of[s] == c;
+      for (int cur = c; !has;) {   // walk the cycle through c
+        int s = 0;
+        while (cta_of[s] >= 0 || (at[bx[s]] != cur && at[by[s]] != cur)) ++s;
+        cta_of[s] = cur;
+        cur = at[bx[s]] == cur ? at[by[s]] : at[bx[s]];
+        has = cur == c;
+      }
+    }
+    for (int s = 0; s < C; ++s) {
+      slot_of[r][cta_of[s]] = (unsigned char)s;
+      at[bx[s]] = at[by[s]] = cta_of[s];
+    }
+  }
+}
+
 bool plan_with_ctas(int n1, int n2, int C, const SliceKnobs& k, SliceShape& sh, size_t& smem) {
   const int max_optin = max_optin_smem();
   sh.rows = n1 < n2 ? 1 : 0;
@@ -53,6 +85,7 @@ bool plan_with_ctas(int n1, int n2, int C, const SliceKnobs& k, SliceShape& sh, 
   sh.block = k.block ? 1 : 0;
   sh.C = C;
   sh.nb = 2 * C;
+  fill_schedule(C, sh.slot_of);
   sh.bs = (sh.nv + sh.nb - 1) / sh.nb;
   if (sh.block) {
     // block form: rows of the vector's 4-entry chunks (and its V entries), no lane layout;

@@ -31,12 +31,13 @@
 // Work split.  A slice is owned by a thread-block cluster of C CTAs (C = 1, 2, 4, 8).  Its
 // vectors form nb = 2C blocks of bs vectors (zero vectors pad the last block); a sweep is a
 // round-robin tournament of the blocks: in block round r CTA c holds the pair of blocks of
-// slot c of the circle method.  Round 0 rotates every vector pair inside the two blocks,
-// later rounds only the bs x bs cross pairs, so each vector pair meets once per sweep.
+// one slot of the circle method (slot c in round 0, later slot_of[r][c]).  Round 0 rotates
+// every vector pair inside the two blocks, later rounds only the bs x bs cross pairs, so each
+// vector pair meets once per sweep.
 // Inside a CTA the pairs of a local round are disjoint and run concurrently, G lanes per
 // pair (32/G pairs per warp), with the inner products reduced by shuffles inside the group.
-// Between block rounds the CTAs trade blocks through a double-buffered global buffer (one
-// cluster barrier per exchange).  For the rebuild the CTAs pool their kept vectors in the
+// Between block rounds each CTA keeps one block and trades the other through a double-buffered
+// global buffer (one cluster barrier per exchange).  For the rebuild the CTAs pool their kept vectors in the
 // exchange buffer (in cluster-rank order) and each CTA writes D_tau(B) for 1/C of the
 // columns from all of them: every entry is summed in a fixed order (deterministic) and no
 // CTA writes a partial slice.
@@ -60,6 +61,8 @@ namespace cg = cooperative_groups;
 
 namespace tsvd {
 
+constexpr int kMaxCtasPerSlice = 8;
+
 // The plan of a slice-SVT launch.
 struct SliceShape {
   int nv;     // number of vectors
@@ -76,6 +79,9 @@ struct SliceShape {
   int C;      // CTAs per slice (cluster size)
   int nb;     // vector blocks = 2C
   int bs;     // vectors per block
+  // block schedule: in block round r CTA c of the cluster holds the pair of circle slot
+  // slot_of[r][c] (fill_schedule), so that one of its blocks stays where it is between rounds
+  unsigned char slot_of[2 * kMaxCtasPerSlice - 1][kMaxCtasPerSlice];
   int kcap;   // kept vectors per rebuild group: 2 bs, or as many rows of ld floats as the
               // 2 bs rows of rowp floats hold (a cluster's U-form rebuild imports those)
   size_t xbuf_floats;   // exchange buffer per slice (floats)
@@ -388,8 +394,8 @@ __device__ __forceinline__ int jacobi_pairs(float* __restrict__ Wr, float* __res
 template <int G, int CPL, int NP>
 __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __restrict__ Wi,
                                             int rowp, int nchunkv, int bs, int nv, int vx0,
-                                            int vy0, int group, int ngroups, int gl, float tol2,
-                                            float floor2, float big2) {
+                                            int vy0, int xrow, int yrow, int group, int ngroups,
+                                            int gl, float tol2, float floor2, float big2) {
   constexpr bool kVRes = CPL * NP <= 3;
   constexpr int CV = kVRes ? CPL : 1;   // nv <= len: a vector has at most CPL V chunks a lane
   float4 xr[NP][CPL], xi[NP][CPL], vxr[NP][CV], vxi[NP][CV];
@@ -401,7 +407,7 @@ __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __res
     slot[i] = group + i * ngroups;
     has[i] = slot[i] < bs && vx0 + slot[i] < nv;
     dirty[i] = false;
-    const int p = has[i] ? slot[i] : 0;
+    const int p = xrow + (has[i] ? slot[i] : 0);
     const float4* xr4 = reinterpret_cast<const float4*>(Wr + p * rowp);
     const float4* xi4 = reinterpret_cast<const float4*>(Wi + p * rowp);
 #pragma unroll
@@ -432,7 +438,7 @@ __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __res
       int y = slot[i] + lr;
       if (y >= bs) y -= bs;
       real[i] = has[i] && (all || vy0 + y < nv);
-      q[i] = has[i] ? bs + y : 1;
+      q[i] = yrow + (has[i] ? y : 0);
       any |= real[i];
     }
     // every lane of the warp takes part in the shuffles when any group has work
@@ -480,8 +486,8 @@ __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __res
               yi4[c] = vyi;
             }
         } else {
-          float4* xr4 = reinterpret_cast<float4*>(Wr + slot[i] * rowp);
-          float4* xi4 = reinterpret_cast<float4*>(Wi + slot[i] * rowp);
+          float4* xr4 = reinterpret_cast<float4*>(Wr + (xrow + slot[i]) * rowp);
+          float4* xi4 = reinterpret_cast<float4*>(Wi + (xrow + slot[i]) * rowp);
           for (int u = 0; u < ncv; ++u) {
             const int c = G * CPL + gl + G * u;
             float4 ar = xr4[c], ai = xi4[c], vyr = yr4[c], vyi = yi4[c];
@@ -501,8 +507,8 @@ __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __res
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     if (!dirty[i]) continue;
-    float4* xr4 = reinterpret_cast<float4*>(Wr + slot[i] * rowp);
-    float4* xi4 = reinterpret_cast<float4*>(Wi + slot[i] * rowp);
+    float4* xr4 = reinterpret_cast<float4*>(Wr + (xrow + slot[i]) * rowp);
+    float4* xi4 = reinterpret_cast<float4*>(Wi + (xrow + slot[i]) * rowp);
 #pragma unroll
     for (int u = 0; u < CPL; ++u) {
       xr4[gl + G * u] = xr[i][u];
@@ -588,25 +594,25 @@ __device__ __forceinline__ float* xblock(float* xbuf, const SliceShape& sh, int 
   return xbuf + (((size_t)par * sh.nb + blk) * 2 + plane) * (size_t)sh.bs * sh.rowp;
 }
 
-// The CTA's two blocks (both planes of local slots 0 and 1) to their places bx, by of the exchange
-// buffer, and the blocks bx, by of the buffer into the slots: four 128-bit streams a thread, the
-// imports asynchronous (all of a thread's in flight at once, past L1).  The cluster barrier
-// between the two is the release and the acquire they need.  Bound by L2 latency: one
-// round trip each way instead of four, and no device-wide fence (9 slices of 32 x 32 on 8 CTAs
-// each: 0.75 -> 0.40 ms a t-SVT; 31 slices of 240 x 320: 6.3 -> 6.0 ms).
-__device__ void export_blocks(float* xbuf, const SliceShape& sh, int par, int bx, int by,
-                              const float* Wr, const float* Wi) {
+// Block `blk`, held in local rows row0 .. row0 + bs - 1 (both planes), to its place in the exchange
+// buffer, and back: two 128-bit streams a thread, the imports asynchronous (all of a thread's
+// in flight at once, past L1).  The cluster barrier between an export and the imports is the
+// release and the acquire they need.  Bound by L2, through which a block passes twice, at about
+// 9 TB/s over the chip: with the device-wide fence and the four round trips of the first form
+// gone (9 slices of 32 x 32 on 8 CTAs each: 0.75 -> 0.40 ms a t-SVT), a CTA that traded both of
+// its blocks still spent 12400 cycles an exchange on 70 KB blocks, 29% of its time; with one
+// block staying (fill_schedule) 31 slices of 240 x 320 take 5.7 ms a t-SVT instead of 6.0, 51
+// of 144 x 176 1.74 instead of 1.86.
+__device__ void export_block(float* xbuf, const SliceShape& sh, int par, int blk, const float* Wr,
+                             const float* Wi, int row0) {
   const int n4 = sh.bs * sh.rowp / 4;
-  const float4* r4 = reinterpret_cast<const float4*>(Wr);
-  const float4* i4 = reinterpret_cast<const float4*>(Wi);
-  float4* x4 = reinterpret_cast<float4*>(xblock(xbuf, sh, par, bx, 0));
-  float4* y4 = reinterpret_cast<float4*>(xblock(xbuf, sh, par, by, 0));
-#pragma unroll 2
+  const float4* r4 = reinterpret_cast<const float4*>(Wr + (size_t)row0 * sh.rowp);
+  const float4* i4 = reinterpret_cast<const float4*>(Wi + (size_t)row0 * sh.rowp);
+  float4* x4 = reinterpret_cast<float4*>(xblock(xbuf, sh, par, blk, 0));
+#pragma unroll 4
   for (int i = threadIdx.x; i < n4; i += blockDim.x) {
     x4[i] = r4[i];
     x4[n4 + i] = i4[i];
-    y4[i] = r4[n4 + i];
-    y4[n4 + i] = i4[n4 + i];
   }
 }
 
@@ -615,21 +621,19 @@ __device__ __forceinline__ void copy_async16(float4* dst, const float4* src) {
                :: "r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
-__device__ void import_blocks(float* xbuf, const SliceShape& sh, int par, int bx, int by, float* Wr,
-                              float* Wi) {
+// Started here, finished by import_wait().
+__device__ void import_block(float* xbuf, const SliceShape& sh, int par, int blk, float* Wr,
+                             float* Wi, int row0) {
   const int n4 = sh.bs * sh.rowp / 4;
-  float4* r4 = reinterpret_cast<float4*>(Wr);
-  float4* i4 = reinterpret_cast<float4*>(Wi);
-  const float4* x4 = reinterpret_cast<const float4*>(xblock(xbuf, sh, par, bx, 0));
-  const float4* y4 = reinterpret_cast<const float4*>(xblock(xbuf, sh, par, by, 0));
+  float4* r4 = reinterpret_cast<float4*>(Wr + (size_t)row0 * sh.rowp);
+  float4* i4 = reinterpret_cast<float4*>(Wi + (size_t)row0 * sh.rowp);
+  const float4* x4 = reinterpret_cast<const float4*>(xblock(xbuf, sh, par, blk, 0));
   for (int i = threadIdx.x; i < n4; i += blockDim.x) {
     copy_async16(r4 + i, x4 + i);
     copy_async16(i4 + i, x4 + n4 + i);
-    copy_async16(r4 + n4 + i, y4 + i);
-    copy_async16(i4 + n4 + i, y4 + n4 + i);
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
 }
+__device__ __forceinline__ void import_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Global index of entry p of column c of B (the slice in vector orientation).
 __device__ __forceinline__ size_t b_index(const SliceShape& sh, int n1, int p, int c) {
@@ -1065,22 +1069,25 @@ __device__ void svt_slice(const SliceArgs& a, const SliceShape& sh, int so, int 
   }
   const int trips = (bs + ngroups - 1) / ngroups;
   int sweeps = 0, converged = 0, par = 0;
+  int xrow = 0, yrow = bs;   // where the x and the y block of the round are held
   for (int sw = 0; sw < a.max_sweeps; ++sw) {
     int rotated = 0;
     for (int r = 0; r < nb - 1; ++r) {
-      round_robin_pair(r, crank, nb, bx, by);
+      round_robin_pair(r, sh.slot_of[r][crank], nb, bx, by);
       const int vx0 = bx * bs, vy0 = by * bs;
       const int nlr = sh.block ? 0 : (r == 0 ? nl - 1 : bs);   // local rounds (pairwise form)
       if (sh.block) {
         block_gram(Wr, Wi, rowp, (len + 3) / 4, nl, bsm);
         __syncthreads();
-        rotated |= block_inner(bsm, sh, r, bx, by, tol2, floor2, big2);
+        // (the local rows in the order they are held)
+        rotated |= block_inner(bsm, sh, r, xrow == 0 ? bx : by, xrow == 0 ? by : bx, tol2, floor2,
+                               big2);
         block_update(Wr, Wi, rowp, rowp / 4, nl, bsm);
         __syncthreads();
       }
       if (r > 0 && nlr > 0 && trips <= NP)
-        rotated |= cross_rounds<G, CPL, NP>(Wr, Wi, rowp, nchunkv, bs, sh.nv, vx0, vy0, group,
-                                            ngroups, gl, tol2, floor2, big2);
+        rotated |= cross_rounds<G, CPL, NP>(Wr, Wi, rowp, nchunkv, bs, sh.nv, vx0, vy0, xrow, yrow,
+                                            group, ngroups, gl, tol2, floor2, big2);
       else for (int lr = 0; lr < nlr; ++lr) {
         for (int k0 = 0; k0 < trips; k0 += NP) {
           int p[NP], q[NP];
@@ -1099,6 +1106,10 @@ __device__ void svt_slice(const SliceArgs& a, const SliceShape& sh, int so, int 
               rp = gp < sh.nv && gq < sh.nv;
             }
             real[i] = rp;
+            if (r > 0) {   // pp < bs <= qq: where the blocks are held (round 0: x, then y)
+              pp += xrow;
+              qq += yrow - bs;
+            }
             p[i] = rp ? pp : 0;
             q[i] = rp ? qq : 1;
             any_real |= rp;
@@ -1115,13 +1126,30 @@ __device__ void svt_slice(const SliceArgs& a, const SliceShape& sh, int so, int 
       if (sweep_end)
         local_any = (__syncthreads_or(rotated & 1) ? 1 : 0) | (__syncthreads_or(rotated & 2) ? 2 : 0);
       if (C > 1) {
-        // trade blocks: write both, barrier, read the next round's pair
+        // trade blocks: write, barrier, read
         if (sweep_end && tid == 0) s_flag[sw & 1] = local_any;
-        export_blocks(xbuf, sh, par, bx, by, Wr, Wi);
-        cluster.sync();
-        int nbx, nby;
-        round_robin_pair(sweep_end ? 0 : r + 1, crank, nb, nbx, nby);
-        import_blocks(xbuf, sh, par, nbx, nby, Wr, Wi);
+        if (sweep_end) {   // back to circle slot crank, x in the first rows
+          export_block(xbuf, sh, par, bx, Wr, Wi, xrow);
+          export_block(xbuf, sh, par, by, Wr, Wi, yrow);
+          cluster.sync();
+          round_robin_pair(0, crank, nb, bx, by);
+          xrow = 0;
+          yrow = bs;
+          import_block(xbuf, sh, par, bx, Wr, Wi, xrow);
+          import_block(xbuf, sh, par, by, Wr, Wi, yrow);
+        } else {           // one block stays, the other is traded
+          int nbx, nby;
+          round_robin_pair(r + 1, sh.slot_of[r + 1][crank], nb, nbx, nby);
+          const bool keep_x = nbx == bx || nby == bx;   // else the old y stays
+          const int stay = keep_x ? xrow : yrow, go = keep_x ? yrow : xrow;
+          const bool stay_is_x = nbx == (keep_x ? bx : by);
+          export_block(xbuf, sh, par, keep_x ? by : bx, Wr, Wi, go);
+          cluster.sync();
+          import_block(xbuf, sh, par, stay_is_x ? nby : nbx, Wr, Wi, go);
+          xrow = stay_is_x ? stay : go;
+          yrow = stay_is_x ? go : stay;
+        }
+        import_wait();
         par ^= 1;
         if (sweep_end) {
           int any = 0;
