@@ -97,10 +97,10 @@ WORKLOADS = {
 # the current source, so its roofline reports none.
 TUBE_TRAFFIC = {"workload": "color",
                 "sources": {"paper_1407_1785_gb300/csrc/tube_tile.cuh":
-                            "0200a606ff6e438f8f86a5486581e4bdb0c500caa8365b9a944d2c87be1e8b8b",
+                            "4cd354311943b15da7435ae87d3f5fd55e228ea7f8302717ee07152143564749",
                             "paper_1407_1785_gb300/csrc/tube_pass.cu":
                             "c8db9e21a8ca9b2ac2529373ff872fb62320ae3fa533fc2a30f6ed4348e14291"},
-                "bytes_per_launch": 219881472 + 106778624}
+                "bytes_per_launch": 219901696 + 102524416}
 
 
 def tube_traffic(workload):
