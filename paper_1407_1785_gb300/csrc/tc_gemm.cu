@@ -149,11 +149,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-// Asynchronous global -> shared copies of 8 and 16 bytes, of which `bytes` are read and the rest
-// written as zeros.
-__device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(bytes)
+// Asynchronous global -> shared copies of 8 bytes, and of 16 bytes of which `bytes` (8 or 16) are
+// read and the rest written as zeros; both addresses aligned to the copy.
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
                : "memory");
 }
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
@@ -295,8 +294,8 @@ struct Share {
   // Asynchronous copy of the chunk at l0 into the thread's raw slots, pairs of entries at
   // raw[(u EPC / 2 + q / 2) NCONV + tid]: the thread that converts an entry is the one that
   // copied it, so the copies need no barrier, only the thread's own cp.async.wait_group.
-  // `any`: an address that can be read (entries past K copy nothing from it).
-  __device__ __forceinline__ void issue(float4* raw, int l0, int K, const float2* any) {
+  // Entries past K are stored as zeros: a copy of no bytes would need an aligned source too.
+  __device__ __forceinline__ void issue(float4* raw, int l0, int K) {
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       if (off[u] < 0) continue;
@@ -304,12 +303,15 @@ struct Share {
 #pragma unroll
       for (int q = 0; q < C::EPC; q += 2) {
         float4* dst = raw + (size_t)(u * C::EPC + q) / 2 * NCONV + threadIdx.x;
-        if (vec[u]) {
-          cp_async16(dst, q < left ? src[u] + q : any, max(0, min(2, left - q)) * 8);
+        float2* d2 = reinterpret_cast<float2*>(dst);
+        if (q >= left) {
+          *dst = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else if (vec[u]) {
+          cp_async16(dst, src[u] + q, q + 1 < left ? 16 : 8);
         } else {
-          float2* d2 = reinterpret_cast<float2*>(dst);
-          cp_async8(d2, q < left ? src[u] + q * sl[u] : any, q < left ? 8 : 0);
-          cp_async8(d2 + 1, q + 1 < left ? src[u] + (q + 1) * sl[u] : any, q + 1 < left ? 8 : 0);
+          cp_async8(d2, src[u] + q * sl[u]);
+          if (q + 1 < left) cp_async8(d2 + 1, src[u] + (q + 1) * sl[u]);
+          else d2[1] = make_float2(0.f, 0.f);
         }
       }
     }
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
       // chunks 0 and 1 in flight before the loop; one commit group per chunk (empty past nk)
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        if (c < nk) sh.issue(raw_of(c), c * C::BK, g.K, A);
+        if (c < nk) sh.issue(raw_of(c), c * C::BK, g.K);
         cp_async_commit();
       }
     }
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
     if (conv) {
       if constexpr (L::RAW_STAGES > 0) {
         // chunk kc + 2 into the slot chunk kc - 1 used (converted by this thread last time)
-        if (kc + 2 < nk) sh.issue(raw_of(kc + 2), (kc + 2) * C::BK, g.K, A);
+        if (kc + 2 < nk) sh.issue(raw_of(kc + 2), (kc + 2) * C::BK, g.K);
         cp_async_commit();
       }
       // the MMAs of chunk kc - 2 have read this buffer
