@@ -166,32 +166,36 @@ __device__ bool batch_tube_args(const BatchDesc& d, const BatchIter& it, TubeArg
   return true;
 }
 
+// Without cross_rounds: their resident vectors, inlined for every chunk count beside the tube
+// tiles, spilled 1.8 KB a thread (0.7 without), and an iteration waits for its slowest slice.
+// 15 iterations, ms: 4 tensors up to 144 x 176 x 30 and 96 x 128 x 100 34.5 -> 29.0; 6 up to
+// 96 x 90 x 30 10.3 -> 9.5.
 template <int CMAX>
 __device__ void batch_slice(const SliceArgs& a, const SliceShape& sh, int so, int crank,
                             float* xbuf, unsigned char* smem_raw, SliceShared& ss) {
   switch (sh.cpl) {
-    case 1: svt_slice<kBatchG, 1, 1>(a, sh, so, crank, xbuf, smem_raw, ss); break;
+    case 1: svt_slice<kBatchG, 1, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss); break;
     case 2:
-      if constexpr (CMAX >= 2) svt_slice<kBatchG, 2, 1>(a, sh, so, crank, xbuf, smem_raw, ss);
+      if constexpr (CMAX >= 2) svt_slice<kBatchG, 2, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss);
       break;
     case 3:
-      if constexpr (CMAX >= 3) svt_slice<kBatchG, 3, 1>(a, sh, so, crank, xbuf, smem_raw, ss);
+      if constexpr (CMAX >= 3) svt_slice<kBatchG, 3, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss);
       break;
     case 4:
-      if constexpr (CMAX >= 4) svt_slice<kBatchG, 4, 1>(a, sh, so, crank, xbuf, smem_raw, ss);
+      if constexpr (CMAX >= 4) svt_slice<kBatchG, 4, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss);
       break;
     case 6:
-      if constexpr (CMAX >= 6) svt_slice<kBatchG, 6, 1>(a, sh, so, crank, xbuf, smem_raw, ss);
+      if constexpr (CMAX >= 6) svt_slice<kBatchG, 6, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss);
       break;
     case 8:
-      if constexpr (CMAX >= 8) svt_slice<kBatchG, 8, 1>(a, sh, so, crank, xbuf, smem_raw, ss);
+      if constexpr (CMAX >= 8) svt_slice<kBatchG, 8, 1, false>(a, sh, so, crank, xbuf, smem_raw, ss);
       break;
     default: break;
   }
 }
 
 template <int CMAX>
-__global__ void __maxnreg__(max_regs_for(CMAX)) batch_iter_kernel(BatchLaunch L) {
+__global__ void __maxnreg__(max_regs_for(CMAX, false)) batch_iter_kernel(BatchLaunch L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ SliceShared ss;
   __shared__ int s_item;
@@ -356,7 +360,7 @@ bool batch_plan(const BatchTensor* ts, int n, int C, int small_nv, BatchPlan& pl
     if (sh.C > 1) plan.xbuf_floats = std::max(plan.xbuf_floats, sh.xbuf_floats);
   }
   plan.cmax = cmax <= 4 ? 4 : 8;   // (a 2-chunk instance would run at 80 registers and spill)
-  plan.threads = max_warps_for(plan.cmax) * 32;
+  plan.threads = max_warps_for(plan.cmax, false) * 32;
   if (plan.threads < TILE_THREADS) return false;
   plan.smem = smem;
   if (smem + kStaticSmemReserve > (size_t)max_optin_smem()) return false;

@@ -6,7 +6,7 @@ namespace tsvd {
 namespace {
 
 template <int G, int CPL, int NP>
-__global__ void __maxnreg__(max_regs_for(CPL * NP))
+__global__ void __maxnreg__(max_regs_for(CPL * NP, true))
     jacobi_svt_kernel(SliceArgs a, SliceShape sh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ SliceShared ss;
@@ -16,7 +16,7 @@ __global__ void __maxnreg__(max_regs_for(CPL * NP))
   float* xbuf = C > 1 ? reinterpret_cast<float*>(static_cast<char*>(a.scratch) +
                                                  (size_t)so * sh.xbuf_floats * sizeof(float))
                       : nullptr;
-  svt_slice<G, CPL, NP>(a, sh, so, crank, xbuf, smem_raw, ss);
+  svt_slice<G, CPL, NP, true>(a, sh, so, crank, xbuf, smem_raw, ss);
 }
 
 template <int G, int CPL, int NP>

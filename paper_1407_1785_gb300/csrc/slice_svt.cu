@@ -238,7 +238,7 @@ cudaError_t launch_jacobi_svt(const SliceArgs& a, cudaStream_t st) {
     return cudaErrorInvalidValue;
   const int gpw = 32 / sh.G;
   const int per_warp = gpw * sh.np;           // pairs a warp has in flight
-  const int maxw = max_warps_for(sh.cpl * sh.np);
+  const int maxw = max_warps_for(sh.cpl * sh.np, true);
   // enough groups for all pairs of a local round in as few passes as fit, balanced
   const int passes = (sh.bs + maxw * per_warp - 1) / (maxw * per_warp);
   int nwarps = (sh.bs + passes * per_warp - 1) / (passes * per_warp);

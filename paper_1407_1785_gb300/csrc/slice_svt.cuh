@@ -527,11 +527,12 @@ __device__ __forceinline__ int cross_rounds(float* __restrict__ Wr, float* __res
   return flags;
 }
 
-// Largest CTA for a chunk count: the pair registers (16 floats per chunk, 8 more with a V part
-// that stays) must fit.  `chunks` = chunks per lane x pairs in flight.  128 registers for up to
-// 4 chunks: caps of 80 (up to 2) and 112 (3) spilled them and cost more than the warps gave.
-__host__ __device__ constexpr int max_warps_for(int chunks) {
-  return chunks <= 4 ? 16 : chunks <= 8 ? 12 : 8;
+// Largest CTA for a chunk count: the pair registers (16 floats per chunk) must fit.  `chunks` =
+// chunks per lane x pairs in flight; `xres`: the kernel has cross_rounds, whose resident x and V
+// entries spill under 80 (up to 2 chunks) and 112 registers (3).
+__host__ __device__ constexpr int max_warps_for(int chunks, bool xres) {
+  return chunks <= 2 && !xres ? 24 : chunks == 3 && !xres ? 18
+       : chunks <= 4 ? 16 : chunks <= 8 ? 12 : 8;
 }
 
 // Copy block `blk` of the slice (vectors blk*bs .. blk*bs+bs-1, zero past nv) into local
@@ -642,10 +643,10 @@ __device__ __forceinline__ size_t b_index(const SliceShape& sh, int n1, int p, i
 
 // Register budget of a thread: the register file over the largest CTA for a chunk count
 // (the launch trims the CTA when the allocation granularity leaves fewer threads).
-__host__ __device__ constexpr int max_regs_for(int chunks) {
-  return (65536 / (max_warps_for(chunks) * 32)) / 8 * 8 > 255
+__host__ __device__ constexpr int max_regs_for(int chunks, bool xres) {
+  return (65536 / (max_warps_for(chunks, xres) * 32)) / 8 * 8 > 255
              ? 255
-             : (65536 / (max_warps_for(chunks) * 32)) / 8 * 8;
+             : (65536 / (max_warps_for(chunks, xres) * 32)) / 8 * 8;
 }
 
 // Shared-memory scalars of one slice SVT (static __shared__ in the kernels: the same offset
@@ -983,7 +984,8 @@ __device__ void block_update(float* __restrict__ Xr, float* __restrict__ Xi, int
 // cluster's block-exchange buffer xbuf (C > 1) and the CTA's dynamic shared memory smem_raw.
 // With a.prerot (V form, a.vin set) the initial vectors are B V / V^T B computed from the
 // slice B = a.ahat itself (load_blocks_rotated) rather than read from a pre-rotated input.
-template <int G, int CPL, int NP>
+// XRES: cross rounds keep x in registers where one pass of the groups covers a round.
+template <int G, int CPL, int NP, bool XRES>
 __device__ void svt_slice(const SliceArgs& a, const SliceShape& sh, int so, int crank,
                           float* xbuf, unsigned char* smem_raw, SliceShared& ss) {
   const int len = sh.len, ld = sh.ld, rowp = sh.rowp, nc = sh.nc, bs = sh.bs, nb = sh.nb;
@@ -1085,7 +1087,7 @@ __device__ void svt_slice(const SliceArgs& a, const SliceShape& sh, int so, int 
         block_update(Wr, Wi, rowp, rowp / 4, nl, bsm);
         __syncthreads();
       }
-      if (r > 0 && nlr > 0 && trips <= NP)
+      if (XRES && r > 0 && nlr > 0 && trips <= NP)
         rotated |= cross_rounds<G, CPL, NP>(Wr, Wi, rowp, nchunkv, bs, sh.nv, vx0, vy0, xrow, yrow,
                                             group, ngroups, gl, tol2, floor2, big2);
       else for (int lr = 0; lr < nlr; ++lr) {
