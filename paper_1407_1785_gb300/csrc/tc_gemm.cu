@@ -29,7 +29,11 @@
 // moves 120 KB through staging, ~1800 cycles at 128 B a cycle, of which a chunk now takes 2400.
 // With 256 threads that also issued the MMAs (18 x 64 cycles in front of one warp's conversion)
 // and staged whole tiles a chunk took 3100 (us, M x N x K, batch): 40 x 40 x 320, 31: 41 -> 27;
-// 320 x 40 x 240, 31: 31 -> 27; 352 x 80 x 288, 91: 146 -> 121; TF32 156 -> 96, BF16 128 -> 72.
+// 320 x 40 x 240, 31: 31 -> 27; 352 x 80 x 288, 91: 146 -> 121.  TF32 and BF16 load through
+// registers, 16 bytes at a time where K is contiguous: 352 x 80 x 288, 91, B along K: TF32 155 ->
+// 87, BF16 125 -> 62; A and B along K: TF32 169 -> 110, BF16 143 -> 87.  With one chunk the
+// prologue counts: the first chunk is staged while the last warp allocates, and no MMA is issued
+// for K past the operands (300 x 300 x 8, 31, TF32 21.4 -> 19.6, 3XTF32 20.3 -> 18.5).
 //
 // Every mbarrier wait is bounded; on expiry the kernel counts a timeout (read by the host
 // through tc_gemm_take_timeouts), waits again (bounded) for its own MMAs, frees its tensor
@@ -238,12 +242,15 @@ struct Share {
   __device__ __forceinline__ void init(const CGemm& g, const float2* A, const float2* B, int i0,
                                        int j0) {
     const int ra = min(BM, g.M - i0), rb = min(BN, g.N - j0);
+    const float ira = __frcp_rn((float)ra), irb = __frcp_rn((float)rb);
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       int item = threadIdx.x + NCONV * u;
       const bool is_a = item < ra * L::KG;
       if (!is_a) item -= ra * L::KG;
-      const int rows = is_a ? ra : rb, kg = item / rows, r = item - kg * rows;
+      const int rows = is_a ? ra : rb;
+      // item / rows: (item + 1/2) / rows is at least 1/256 from a whole number and below 2^11
+      const int kg = (int)(((float)item + 0.5f) * (is_a ? ira : irb)), r = item - kg * rows;
       k0[u] = kg * C::EPC;
       sl[u] = is_a ? g.a.s1 : g.b.s0;
       conj[u] = (is_a ? g.a.conj : g.b.conj) != 0;
@@ -281,14 +288,23 @@ struct Share {
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int left = off[u] < 0 ? 0 : K - l0 - k0[u];
+      if (vec[u] && left >= C::EPC) {
 #pragma unroll
-      for (int q = 0; q < C::EPC; ++q)
-        x[u][q] = q < left ? src[u][q * sl[u]] : make_float2(0.f, 0.f);
+        for (int q = 0; q < C::EPC; q += 2) {
+          const float4 v = *reinterpret_cast<const float4*>(src[u] + q);
+          x[u][q] = make_float2(v.x, v.y);
+          x[u][q + 1] = make_float2(v.z, v.w);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < C::EPC; ++q)
+          x[u][q] = q < left ? src[u][q * sl[u]] : make_float2(0.f, 0.f);
+      }
     }
     advance();
 #pragma unroll
-    for (int u = 0; u < PER; ++u)
-      if (off[u] >= 0) store(u, x[u], stage);
+    for (int u = 0; u < PER; ++u)   // (entries past the last instruction's K are not read)
+      if (off[u] >= 0 && l0 + k0[u] / C::KMMA * C::KMMA < K) store(u, x[u], stage);
   }
 
   // Asynchronous copy of the chunk at l0 into the thread's raw slots, pairs of entries at
@@ -372,21 +388,21 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   auto raw_of = [&](int c) { return raw + (size_t)(c % 3) * ((L::RAW_A + L::RAW_B) / 16); };
   const uint32_t bar0 = smem_u32(&bars[0]), bar1 = smem_u32(&bars[1]);
 
-  if (warp == 0) {
+  // The issuing warp allocates while the others already stage the first chunks; the barrier of
+  // chunk 0 publishes the tensor memory's address and the mbarriers.
+  const bool conv = tid < NCONV;   // the last warp issues the MMAs
+  if (!conv) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    if (lane == 0) {
+      mbar_init(bar0);
+      mbar_init(bar1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
-  if (tid == 0) {
-    mbar_init(bar0);
-    mbar_init(bar1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
 
   // columns of the instruction: those the tile has, in steps of 16
   const int ncol = min(BN, (g.N - j0 + 15) / 16 * 16);
@@ -396,7 +412,6 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   constexpr int KSTEPS = C::BK / C::KMMA;
   const int nk = (g.K + C::BK - 1) / C::BK;
   bool timed_out = false;
-  const bool conv = tid < NCONV;   // the last warp issues the MMAs
   Share<ENG> sh;
   if (conv) {
     sh.init(g, A, B, i0, j0);
@@ -438,24 +453,31 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
     }
     if (tid == NCONV) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t tmem = *tmem_slot;
       const uint32_t a_base = smem_u32(st), b_base = a_base + L::NPLANE * L::PLANE_A;
+      auto step = [&](int p, int s) {
 #pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        const uint32_t d = tmem + (uint32_t)(p * BN);
-#pragma unroll
-        for (int s = 0; s < KSTEPS; ++s) {
-#pragma unroll
-          for (int t = 0; t < (C::NSPLIT == 2 ? 3 : 1); ++t) {
-            // 3XTF32 terms: (hi, hi), (hi, lo), (lo, hi)
-            const int ha = t == 2 ? 1 : 0, hb = t == 1 ? 1 : 0;
-            const uint32_t aa = a_base + (uint32_t)((p * C::NSPLIT + ha) * L::PLANE_A) +
-                                (uint32_t)(s * 2) * LBO_A;
-            const uint32_t bb = b_base + (uint32_t)((p * C::NSPLIT + hb) * L::PLANE_B) +
-                                (uint32_t)(s * 2) * LBO_B;
-            const uint32_t acc = (kc > 0 || s > 0 || t > 0) ? 1u : 0u;
-            mma<ENG>(d, sdesc(aa, LBO_A, SBO), sdesc(bb, LBO_B, SBO), idesc, acc);
-          }
+        for (int t = 0; t < (C::NSPLIT == 2 ? 3 : 1); ++t) {
+          // 3XTF32 terms: (hi, hi), (hi, lo), (lo, hi)
+          const int ha = t == 2 ? 1 : 0, hb = t == 1 ? 1 : 0;
+          const uint32_t aa = a_base + (uint32_t)((p * C::NSPLIT + ha) * L::PLANE_A) +
+                              (uint32_t)(s * 2) * LBO_A;
+          const uint32_t bb = b_base + (uint32_t)((p * C::NSPLIT + hb) * L::PLANE_B) +
+                              (uint32_t)(s * 2) * LBO_B;
+          const uint32_t acc = (kc > 0 || s > 0 || t > 0) ? 1u : 0u;
+          mma<ENG>(tmem + (uint32_t)(p * BN), sdesc(aa, LBO_A, SBO), sdesc(bb, LBO_B, SBO), idesc,
+                   acc);
         }
+      };
+      const int left = g.K - kc * C::BK;
+      if (left > C::BK - C::KMMA) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+          for (int s = 0; s < KSTEPS; ++s) step(p, s);
+      } else {   // the rest of the chunk is zeros
+        for (int p = 0; p < 3; ++p)
+          for (int s = 0; s * C::KMMA < left; ++s) step(p, s);
       }
       asm volatile(
           "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -474,6 +496,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   }
   const bool good = !timed_out && !__syncthreads_or(!ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
   if (good && nk > 0 && warp < 8) {   // 4 row groups x 2 halves of the columns
     const int q = warp & 3, half = warp >> 2;
     const int i = i0 + 32 * q + lane;
@@ -504,7 +527,7 @@ __global__ void __launch_bounds__(NTHR, 1) cgemm_tc_kernel(CGemm g) {
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) {
+  if (!conv) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(TMEM_COLS));
