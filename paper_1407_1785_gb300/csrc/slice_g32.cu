@@ -4,7 +4,7 @@
 namespace tsvd {
 
 cudaError_t launch_lanes_32(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
-                           cudaStream_t st) {
+                           bool xres, cudaStream_t st) {
   TSVD_CASE(32, 1, 1)
   TSVD_CASE(32, 2, 1)
   TSVD_CASE(32, 3, 1)

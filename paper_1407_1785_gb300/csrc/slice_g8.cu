@@ -4,7 +4,7 @@
 namespace tsvd {
 
 cudaError_t launch_lanes_8(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
-                           cudaStream_t st) {
+                           bool xres, cudaStream_t st) {
   TSVD_CASE(4, 1, 1)
   TSVD_CASE(4, 2, 1)
   TSVD_CASE(8, 1, 1)

@@ -5,8 +5,8 @@
 namespace tsvd {
 namespace {
 
-template <int G, int CPL, int NP>
-__global__ void __maxnreg__(max_regs_for(CPL * NP, true))
+template <int G, int CPL, int NP, bool XRES>
+__global__ void __maxnreg__(max_regs_for(CPL * NP, XRES))
     jacobi_svt_kernel(SliceArgs a, SliceShape sh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ SliceShared ss;
@@ -16,19 +16,19 @@ __global__ void __maxnreg__(max_regs_for(CPL * NP, true))
   float* xbuf = C > 1 ? reinterpret_cast<float*>(static_cast<char*>(a.scratch) +
                                                  (size_t)so * sh.xbuf_floats * sizeof(float))
                       : nullptr;
-  svt_slice<G, CPL, NP, true>(a, sh, so, crank, xbuf, smem_raw, ss);
+  svt_slice<G, CPL, NP, XRES>(a, sh, so, crank, xbuf, smem_raw, ss);
 }
 
-template <int G, int CPL, int NP>
+template <int G, int CPL, int NP, bool XRES>
 cudaError_t launch_gc(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
                       cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(jacobi_svt_kernel<G, CPL, NP>,
+  cudaError_t e = cudaFuncSetAttribute(jacobi_svt_kernel<G, CPL, NP, XRES>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // the register budget can allow fewer threads than the warp cap: the kernel takes any
   // multiple of 32 (it runs a local round's pairs in as many trips as its groups need)
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, jacobi_svt_kernel<G, CPL, NP>);
+  e = cudaFuncGetAttributes(&fa, jacobi_svt_kernel<G, CPL, NP, XRES>);
   if (e != cudaSuccess) return e;
   if (threads > fa.maxThreadsPerBlock) threads = fa.maxThreadsPerBlock / 32 * 32;
   if (threads < 32) return cudaErrorInvalidConfiguration;
@@ -44,14 +44,16 @@ cudaError_t launch_gc(const SliceArgs& a, const SliceShape& sh, size_t smem, int
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, jacobi_svt_kernel<G, CPL, NP>, a, sh);
+  e = cudaLaunchKernelEx(&cfg, jacobi_svt_kernel<G, CPL, NP, XRES>, a, sh);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-#define TSVD_CASE(G_, C_, N_) \
-  if (sh.G == G_ && sh.cpl == C_ && sh.np == N_) \
-    return launch_gc<G_, C_, N_>(a, sh, smem, threads, st);
+// Past 3 chunks both forms have the same budget, and one instance serves them.
+#define TSVD_CASE(G_, C_, N_)                                                  \
+  if (sh.G == G_ && sh.cpl == C_ && sh.np == N_)                               \
+    return xres ? launch_gc<G_, C_, N_, true>(a, sh, smem, threads, st)        \
+                : launch_gc<G_, C_, N_, (C_ * N_ > 3)>(a, sh, smem, threads, st);
 
 }  // namespace
 }  // namespace tsvd

@@ -236,20 +236,41 @@ cudaError_t launch_jacobi_svt(const SliceArgs& a, cudaStream_t st) {
   if (a.wout && a.wout_stride < (int64_t)a.n1 * a.n2) return cudaErrorInvalidValue;
   if ((a.vin || a.vout) && (!sh.vform || a.vstride < (int64_t)sh.nv * sh.nv))
     return cudaErrorInvalidValue;
-  const int gpw = 32 / sh.G;
-  const int per_warp = gpw * sh.np;           // pairs a warp has in flight
-  const int maxw = max_warps_for(sh.cpl * sh.np, true);
+  const int per_warp = 32 / sh.G * sh.np;     // pairs a warp has in flight
+  const int chunks = sh.cpl * sh.np;
   // enough groups for all pairs of a local round in as few passes as fit, balanced
-  const int passes = (sh.bs + maxw * per_warp - 1) / (maxw * per_warp);
-  int nwarps = (sh.bs + passes * per_warp - 1) / (passes * per_warp);
-  // block form: a warp per 4 local vectors (the Gram tiles and update chunks spread over them)
-  if (sh.block) nwarps = (2 * sh.bs + 3) / 4;
-  if (nwarps < kMinWarps) nwarps = kMinWarps;
-  if (nwarps > maxw) nwarps = maxw;
-  const int threads = nwarps * 32;
-  if (sh.G == 32) return launch_lanes_32(a, sh, smem, threads, st);
-  if (sh.G == 16) return launch_lanes_16(a, sh, smem, threads, st);
-  return launch_lanes_8(a, sh, smem, threads, st);
+  auto passes_of = [&](bool x) {
+    const int most = max_warps_for(chunks, x) * per_warp;
+    return (sh.bs + most - 1) / most;
+  };
+  auto warps_of = [&](bool x) {
+    // block form: a warp per 4 local vectors (the Gram tiles and update chunks spread over them)
+    const int per_pass = passes_of(x) * per_warp;
+    const int n = sh.block ? (2 * sh.bs + 3) / 4 : (sh.bs + per_pass - 1) / per_pass;
+    return std::min(std::max(n, kMinWarps), max_warps_for(chunks, x));
+  };
+  auto waves_of = [&](bool x) {
+    const int by_regs = 65536 / (max_regs_for(chunks, x) * warps_of(x) * 32);
+    const int by_smem = (int)(kSmSmem / (smem + kStaticSmemReserve));
+    const int64_t held = (int64_t)device_sm_count() * std::max(1, std::min(by_regs, by_smem));
+    return ((int64_t)a.nslices * sh.C + held - 1) / held;
+  };
+  // Which instance (up to 3 chunks; others have one): the one with x in registers, unless its
+  // 16 warps need two passes a round where 24 (18 at 3 chunks) need one, its registers cost a
+  // wave of CTAs, or there are no cross rounds (C = 1) and the other does not spill (3 chunks).
+  // A t-SVT without / with x in registers, us: two passes, 101 slices of 70 x 90, C = 1: 960 /
+  // 1195; 126 of 80 x 100, 32 lanes, C = 2: 1734 / 1984; a wave, 126 of 80 x 100, 16 lanes,
+  // C = 2: 1071 / 1440; 51 of 96 x 128, 32 lanes, C = 8: 1079 / 1485; 3 chunks, 32 of 61 x 75, 8
+  // lanes, C = 1: 598 / 635.  Else 126 of 61 x 75, 16 lanes, C = 4: 750 / 687; 51 of 61 x 75,
+  // 32 lanes, C = 1: 957 / 895; three passes against two, 126 of 96 x 128, 32 lanes, C = 1:
+  // 2319 / 2234.
+  const bool xres = sh.block || chunks > 3 ||
+                    !(passes_of(true) >= 2 * passes_of(false) || waves_of(false) < waves_of(true) ||
+                      (sh.C == 1 && chunks == 3));
+  const int threads = warps_of(xres) * 32;
+  if (sh.G == 32) return launch_lanes_32(a, sh, smem, threads, xres, st);
+  if (sh.G == 16) return launch_lanes_16(a, sh, smem, threads, xres, st);
+  return launch_lanes_8(a, sh, smem, threads, xres, st);
 }
 
 }  // namespace tsvd

@@ -91,14 +91,19 @@ struct SliceShape {
 
 constexpr int kMinBlock = 16;     // fewest vectors per block before a slice is split further
 constexpr size_t kStaticSmemReserve = 1024;   // static __shared__ of the kernels, with margin
+constexpr size_t kSmSmem = 228 * 1024;        // shared memory of an SM
 
 int max_optin_smem();
 bool plan_with_ctas(int n1, int n2, int C, const SliceKnobs& k, SliceShape& sh, size_t& smem);
 // The kernel instances of one lane count (slice_g8.cu: 4 and 8 lanes a pair, slice_g16.cu,
-// slice_g32.cu); cudaErrorInvalidValue for a plan they do not have.
-cudaError_t launch_lanes_8(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads, cudaStream_t st);
-cudaError_t launch_lanes_16(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads, cudaStream_t st);
-cudaError_t launch_lanes_32(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads, cudaStream_t st);
+// slice_g32.cu); cudaErrorInvalidValue for a plan they do not have.  xres: the instance whose cross
+// rounds keep x in registers (cross_rounds), else the one with more warps for up to 3 chunks.
+cudaError_t launch_lanes_8(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
+                           bool xres, cudaStream_t st);
+cudaError_t launch_lanes_16(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
+                            bool xres, cudaStream_t st);
+cudaError_t launch_lanes_32(const SliceArgs& a, const SliceShape& sh, size_t smem, int threads,
+                            bool xres, cudaStream_t st);
 
 namespace {
 
