@@ -50,20 +50,21 @@ bool pick_group(int ld, int prefer, int& G, int& cpl) {
 // joins two CTAs that hold one of its blocks each, and every CTA holds two blocks, so the next
 // pairs are the edges of cycles over the CTAs; giving each CTA the edge it leaves a cycle by
 // lets every CTA keep one block and trade the other.  The rotations and their order are those
-// of the circle method, whichever CTA does them.  Worked out once per cluster size: a plan is
-// made for every candidate of every launch, and 9 slices of 32 x 32 lost 17 of their 215 us a
-// t-SVT to this walk on the host.
+// of the circle method, whichever CTA does them (in the block form a CTA that holds its y block
+// first takes the pairs of a round in another order).  Worked out by the compiler: a plan is made
+// for every candidate of every launch, and 9 slices of 32 x 32 lost 17 of their 215 us a t-SVT to
+// this walk on the host.
 struct BlockSchedule {
   unsigned char slot_of[2 * kMaxCtasPerSlice - 1][kMaxCtasPerSlice];
 };
 
-static BlockSchedule fill_schedule(int C) {
+constexpr BlockSchedule fill_schedule(int C) {
   BlockSchedule sch = {};
   auto& slot_of = sch.slot_of;
   const int nb = 2 * C;
-  int at[2 * kMaxCtasPerSlice];   // CTA that holds a block
+  int at[2 * kMaxCtasPerSlice] = {};   // CTA that holds a block
   for (int r = 0; r < nb - 1; ++r) {
-    int bx[kMaxCtasPerSlice], by[kMaxCtasPerSlice], cta_of[kMaxCtasPerSlice];
+    int bx[kMaxCtasPerSlice] = {}, by[kMaxCtasPerSlice] = {}, cta_of[kMaxCtasPerSlice] = {};
     for (int s = 0; s < C; ++s) {
       round_robin_pair(r, s, nb, bx[s], by[s]);
       cta_of[s] = r == 0 ? s : -1;
@@ -87,11 +88,36 @@ static BlockSchedule fill_schedule(int C) {
   return sch;
 }
 
-static const BlockSchedule& block_schedule(int C) {
-  static const BlockSchedule of[4] = {fill_schedule(1), fill_schedule(2), fill_schedule(4),
-                                      fill_schedule(8)};
-  return of[C == 8 ? 3 : C / 2];
+// What the exchange of svt_slice relies on: round 0 as loaded (slot c on CTA c), every slot of a
+// round on one CTA, and every CTA with exactly one of its two blocks in the next round (the
+// circle method itself brings every pair of blocks together once).
+constexpr bool one_block_stays(const BlockSchedule& sch, int C) {
+  const int nb = 2 * C;
+  for (int c = 0; c < C; ++c)
+    if (sch.slot_of[0][c] != c) return false;
+  bool met[2 * kMaxCtasPerSlice][2 * kMaxCtasPerSlice] = {};
+  for (int r = 0; r < nb - 1; ++r)
+    for (int c = 0; c < C; ++c) {
+      int bx = 0, by = 0, nx = 0, ny = 0;
+      round_robin_pair(r, sch.slot_of[r][c], nb, bx, by);
+      if (bx == by || met[bx][by] || met[by][bx]) return false;
+      met[bx][by] = true;
+      for (int d = 0; d < c; ++d)
+        if (sch.slot_of[r][d] == sch.slot_of[r][c]) return false;
+      if (r + 2 == nb) continue;
+      round_robin_pair(r + 1, sch.slot_of[r + 1][c], nb, nx, ny);
+      if ((bx == nx || bx == ny) == (by == nx || by == ny)) return false;
+    }
+  return true;
 }
+
+constexpr BlockSchedule kSchedules[4] = {fill_schedule(1), fill_schedule(2), fill_schedule(4),
+                                         fill_schedule(8)};
+static_assert(one_block_stays(kSchedules[0], 1) && one_block_stays(kSchedules[1], 2) &&
+                  one_block_stays(kSchedules[2], 4) && one_block_stays(kSchedules[3], 8),
+              "a CTA must keep one block from round to round");
+
+static const BlockSchedule& block_schedule(int C) { return kSchedules[C == 8 ? 3 : C / 2]; }
 
 bool plan_with_ctas(int n1, int n2, int C, const SliceKnobs& k, SliceShape& sh, size_t& smem) {
   const int max_optin = max_optin_smem();

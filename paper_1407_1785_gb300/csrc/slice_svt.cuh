@@ -125,7 +125,7 @@ __device__ __forceinline__ float group_sum(float v) {
 }
 
 // Pair (p, q) of slot `slot` in round r of the circle method over P (even) players.
-__host__ __device__ inline void round_robin_pair(int r, int slot, int P, int& p, int& q) {
+__host__ __device__ constexpr void round_robin_pair(int r, int slot, int P, int& p, int& q) {
   if (slot == 0) {
     p = P - 1;
     q = r;
