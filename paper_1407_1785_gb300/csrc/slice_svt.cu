@@ -21,7 +21,7 @@ namespace {
 
 // Lanes per pair and 4-entry chunks per lane for vectors of ld floats (a multiple of 4).
 // `prefer` = 0 picks the narrowest group with at most 2 chunks per lane, else 16 lanes;
-// `prefer` = 4, 8 or 16 asks for that group width (more chunks per lane = more independent
+// `prefer` = 4, 8, 16 or 32 asks for that group width (more chunks per lane = more independent
 // work per lane, fewer lanes = fewer shuffle levels and more pairs per warp).
 bool pick_group(int ld, int prefer, int& G, int& cpl) {
   const int nchunk = ld / 4;

@@ -1,7 +1,8 @@
 // tsvd_api.cu -- the C ABI of libtsvd (include/tsvd.h): argument checks, device workspaces,
 // host/device staging and the order of kernel launches of the t-SVT and of the two ADMM
-// solvers.  All arithmetic runs in the kernels of tube_pass.cu and slice_svt.cu; this file
-// only computes the scalar penalty schedule rho_k (Sec. 4 / Sec. 5) on the host.
+// solvers.  All arithmetic runs in the kernels of tube_pass.cu, slice_svt.cuh, rsvt.cu, factor.cu
+// and the products (fp32_gemm.cu, tc_gemm.cu); this file only computes the scalar penalty
+// schedule rho_k (Sec. 4 / Sec. 5) on the host.
 #include "tsvd.h"
 #include "tsvd_internal.h"
 

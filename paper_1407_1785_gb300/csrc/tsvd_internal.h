@@ -202,7 +202,7 @@ cudaError_t launch_jacobi_svt(const SliceArgs& a, cudaStream_t st);
 
 // ---- persistent batched launch (plain form): one kernel launch per ADMM iteration runs the
 // slice SVTs of every tensor of a batch, then the tube passes that follow them, from device
-// work queues (slice_svt.cu).
+// work queues (slice_batch.cu).
 // One tensor of the batch, as the host describes it.
 struct BatchTensor {
   TubeGeom g;
@@ -302,7 +302,7 @@ size_t jacobi_svt_scratch_bytes(int n1, int n2, int nslices, const SliceKnobs& k
 // CTAs per slice the launch would use.
 int jacobi_svt_ctas_per_slice(int n1, int n2, int nslices, const SliceKnobs& k);
 
-// ---- batched complex GEMM with generic strides (rsvt.cu, tc_gemm.cu)
+// ---- batched complex GEMM with generic strides (fp32_gemm.cu, tc_gemm.cu)
 // One operand or the result: entry (i0, i1) of batch entry b at
 // p[(idx ? idx[b] : b) * bs + i0 * s0 + i1 * s1], conjugated when conj.
 struct CMat {
