@@ -291,8 +291,8 @@ cudaError_t launch_jacobi_svt(const SliceArgs& a, cudaStream_t st) {
   // 32 lanes, C = 1: 957 / 895; three passes against two, 126 of 96 x 128, 32 lanes, C = 1:
   // 2319 / 2234.
   const bool xres = sh.block || chunks > 3 ||
-                    !(passes_of(true) >= 2 * passes_of(false) || waves_of(false) < waves_of(true) ||
-                      (sh.C == 1 && chunks == 3));
+                    !(passes_of(true) >= 2 * passes_of(false) || (sh.C == 1 && chunks == 3) ||
+                      (a.nslices * sh.C > device_sm_count() && waves_of(false) < waves_of(true)));
   const int threads = warps_of(xres) * 32;
   if (sh.G == 32) return launch_lanes_32(a, sh, smem, threads, xres, st);
   if (sh.G == 16) return launch_lanes_16(a, sh, smem, threads, xres, st);
